@@ -255,10 +255,10 @@ struct Chol4 {
 // so Phi^T = e_0^T A^-1 B (Eq. 6, p(x_l) = e_0 in the marker-centred basis) is
 //   phi_abc = sum_{i+j+k <= 1 or 2} E_i,a[x] E_j,b[y] E_k,c[z],
 //   E_i,a = n_a P_i(0) P_i(xi_a) / sum_a n_a P_i(xi_a)^2.
-// Nothing is assembled, factored or refined, and no step subtracts nearly
-// equal numbers: offsets are taken from the home-cell centre, where the middle
-// node sits, so the mean offset mu keeps its relative accuracy when the outer
-// weights are tiny (narrow cells between wide ones).  It replaced a 4 x 4 (or
+// Nothing is assembled, factored or refined.  Offsets are taken from the
+// home-cell centre, where the middle node sits, so the mean offset mu keeps its
+// relative accuracy when the outer weights are tiny (narrow cells between wide
+// ones); E_2, a difference of values of order one, keeps its absolute accuracy.  It replaced a 4 x 4 (or
 // 10 x 10) Cholesky solve with a refinement step per marker, which issued 124 M
 // (276 M) warp instructions on 4 M markers at 64 (166) registers; the quadratic
 // build with its interpolation went from 944 to 544 us there, with half the
@@ -271,7 +271,7 @@ template <typename R, int MB>
 struct AxisForm {
   R e0[3], e1[3], e2[MB == 4 ? 1 : 3];
   R m, v, g;      // mean and variance of xi under n, g = m / v
-  R n4[MB == 4 ? 1 : 2];  // quadratic: third and fourth central moments
+  R c3, q2;    // quadratic: third central moment and sum_a n_a P2(xi_a)^2
 };
 
 // Weights relative to the middle node's: w_a / w_1 = exp(-(xi_a^2 - xi_1^2)/eps^2),
@@ -311,8 +311,12 @@ __device__ __forceinline__ bool axis_form(const AxisNodes<R>& s, R inv_eps2, Axi
     f.e2[0] = l0 - f.e0[0] - f.e1[0];
     f.e2[1] = l1 - f.e0[1] - f.e1[1];
     f.e2[2] = l2 - f.e0[2] - f.e1[2];
-    f.n4[0] = nc[0] * c[0] * c[0] + nc[1] * c[1] * c[1] + nc[2] * c[2] * c[2];
-    f.n4[1] = nc[0] * c[0] * c[0] * c[0] + nc[1] * c[1] * c[1] * c[1] + nc[2] * c[2] * c[2] * c[2];
+    f.c3 = nc[0] * c[0] * c[0] + nc[1] * c[1] * c[1] + nc[2] * c[2] * c[2];
+    // The Gram determinant of 1, P1, P2 on three nodes is v sum n P2^2 and also
+    // n_0 n_1 n_2 times the squared Vandermonde determinant.  As c4 - c3^2/v - v^2
+    // the sum would be rounding noise of either sign once an outer weight is tiny.
+    const R vd = s.dm * s.dp * (s.dm + s.dp);
+    f.q2 = (f.e0[0] * vd) * (f.e0[2] * vd) * f.e0[1] * recip(f.v);
   }
   return f.v > (sizeof(R) == 4 ? R(1e-30) : R(1e-290));
 }
@@ -361,23 +365,22 @@ __device__ __forceinline__ R cond1(const AxisForm<R, 4> f[3]) {
 // The same for the quadratic basis, column by column, from the raw moments r_k
 // (k <= 4) of each axis and the monomial coefficients of the orthogonal
 // products: P2 = xi^2 - al xi + be, al = 2 m + s, be = m^2 + s m - v, with
-// s = c3 / v and sum n P2^2 = c4 - s c3 - v^2.
+// s = c3 / v; the fourth central moment is q2 + s c3 + v^2.
 template <typename R>
 __device__ __forceinline__ R cond1(const AxisForm<R, kQuad> f[3]) {
   R r[3][5], iv[3], i2[3], al[3], be[3], m[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const R v = f[d].v, c3 = f[d].n4[0], c4 = f[d].n4[1];
+    const R v = f[d].v, c3 = f[d].c3;
     m[d] = f[d].m;
-    const R mm = m[d] * m[d];
+    iv[d] = recip(v);
+    const R mm = m[d] * m[d], s = c3 * iv[d], c4 = f[d].q2 + s * c3 + v * v;
     r[d][0] = R(1);
     r[d][1] = m[d];
     r[d][2] = v + mm;
     r[d][3] = c3 + m[d] * (R(3) * v + mm);
     r[d][4] = c4 + m[d] * (R(4) * c3 + m[d] * (R(6) * v + mm));
-    iv[d] = recip(v);
-    const R s = c3 * iv[d];
-    i2[d] = recip(c4 - s * c3 - v * v);
+    i2[d] = recip(f[d].q2);
     al[d] = R(2) * m[d] + s;
     be[d] = mm + s * m[d] - v;
 #pragma unroll
@@ -436,25 +439,29 @@ __device__ __forceinline__ R cond_bound(const AxisForm<R, kQuad> f[3]) {
   R q2[3], q4[3], t1[3], t2[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const R v = f[d].v, c3 = f[d].n4[0], c4 = f[d].n4[1], m = f[d].m, mm = m * m, iv = recip(v), s = c3 * iv;
+    const R v = f[d].v, c3 = f[d].c3, m = f[d].m, mm = m * m, iv = recip(v), s = c3 * iv;
     q2[d] = v + mm;
-    q4[d] = c4 + m * (R(4) * c3 + m * (R(6) * v + mm));
+    q4[d] = f[d].q2 + s * c3 + v * v + m * (R(4) * c3 + m * (R(6) * v + mm));
     t1[d] = (R(1) + mm) * iv;
     const R al = R(2) * m + s, be = mm + s * m - v;
-    t2[d] = (R(1) + al * al + be * be) * recip(c4 - s * c3 - v * v);
+    t2[d] = (R(1) + al * al + be * be) * recip(f[d].q2);
   }
   const R ta = R(1) + q2[0] + q2[1] + q2[2] + q4[0] + q4[1] + q4[2] + q2[0] * q2[1] + q2[1] * q2[2] + q2[2] * q2[0];
   const R ti = R(1) + t1[0] + t1[1] + t1[2] + t2[0] + t2[1] + t2[2] + t1[0] * t1[1] + t1[1] * t1[2] + t1[2] * t1[0];
   return R(kQuad) * ta * ti;
 }
 
-// Whether cond_1(A) exceeds `limit` (NaN counts as exceeding).
+// Whether cond_1(A) exceeds `limit`.  NaN counts as exceeding, and so does a
+// norm of P2 that is no normal number (its reciprocal would be infinite, and
+// fmax passes NaN over).
 template <typename R>
 __device__ __forceinline__ bool cond_above(const AxisForm<R, 4> f[3], R limit) {
   return !(cond1(f) <= limit);
 }
 template <typename R>
 __device__ __forceinline__ bool cond_above(const AxisForm<R, kQuad> f[3], R limit) {
+  const R tiny = sizeof(R) == 4 ? R(1e-37) : R(1e-300);
+  if (!(f[0].q2 > tiny && f[1].q2 > tiny && f[2].q2 > tiny)) return true;
   if (cond_bound(f) <= R(0.99) * limit) return false;
   return !(cond1(f) <= limit);
 }
