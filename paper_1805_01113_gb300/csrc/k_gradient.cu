@@ -8,15 +8,70 @@ namespace mls {
 
 template <typename R> constexpr int kGradThreads = sizeof(R) == 4 ? kBlock : kBlockF64;
 
+// One axis of a marker's derivative: the linear basis functions E_0, E_1 and
+// their slopes at the two outer nodes.  E_0 sums to one over the three nodes and
+// the others to zero, so the middle node enters through differences alone.
+template <typename R>
+struct AxisEnds {
+  R e0[2], e1[2], d0[2], d1[2];
+};
+
+// w at the outer nodes against their differences from the middle one.
+template <typename R>
+__device__ __forceinline__ R ends(const R w[2], R lo, R hi) {
+  return w[0] * lo + w[1] * hi;
+}
+
+// The value of node a of three that sum to `sum`, from the outer two.
+template <typename R>
+__device__ __forceinline__ R of_node(const R w[2], R sum, int a) {
+  return a == 0 ? w[0] : a == 2 ? w[1] : sum - w[0] - w[1];
+}
+
+// One component's derivatives as the plain sum over the nodes, where a value of
+// the stencil is not finite (or a difference overflows): an infinity then
+// reaches the derivatives with its own weight's sign only.
+template <typename R, typename FT>
+__device__ __forceinline__ void plain_sum(const AxisEnds<R> f[3], const FT* __restrict__ u, const int xs[3],
+                                          const int rows[3][3], R out[3]) {
+  out[0] = out[1] = out[2] = R(0);
+#pragma unroll 1
+  for (int k = 0; k < 27; ++k) {
+    const int n[3] = {k % 3, k / 3 % 3, k / 9};
+    R e0[3], e1[3], d0[3], d1[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      e0[d] = of_node(f[d].e0, R(1), n[d]);
+      e1[d] = of_node(f[d].e1, R(0), n[d]);
+      d0[d] = of_node(f[d].d0, R(0), n[d]);
+      d1[d] = of_node(f[d].d1, R(0), n[d]);
+    }
+    int o = n[0] == 0 ? xs[0] : n[0] == 1 ? xs[1] : xs[2];
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+      if (q == k / 3) o += rows[q / 3][q % 3];
+    const R v = field_value<R, FT>(u + o);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int a = (d + 1) % 3, b = (d + 2) % 3;
+      out[d] += (d0[d] * (e0[a] * (e0[b] + e1[b]) + e1[a] * e0[b]) + d1[d] * (e0[a] * e0[b])) * v;
+    }
+  }
+}
+
 // G[c][d][l] = sum_k d_d phi_k^l u_c,k.  One thread per marker in tile order.
-// phi_abc = E_0,a k1 + E_1,a k0 (exact_emit), and a derivative along an axis
-// replaces that axis's E by its slopes, so a node takes 6 fused multiply-adds
-// for its three derivatives and 9 for the sums.  Markers without support get
-// G = 0.  The 81 gathers of a marker go through the cache hierarchy (the
-// markers of a home cell are adjacent, so a warp's gathers share lines) and
-// are what the kernel waits for: 286 us on 4 M markers at 64 registers, 291 at
-// 80, 336 at 128, against 38 us for the bytes.  The derivatives from four
-// Cholesky solves, which this form replaced, took 368 us at 128 registers.
+// phi_abc = E_0,a (E_0,b (E_0 + E_1)_c + E_1,b E_0,c) + E_1,a E_0,b E_0,c, and a
+// derivative along an axis replaces that axis's E by its slopes.  The sums are
+// contracted axis by axis over differences between neighbouring nodes, in which
+// a constant part of the field cancels before any rounding: with the field's own
+// values the error of a smooth field grows as its gradient falls, and with the
+// field relative to the home cell's value, rounded per node, a rough one loses.
+// Wave numbers up to 16 per box, error over the gradient's norm, by own values,
+// by home-relative ones and so: 1.4, 1.8 and 1.2e-7 in 48^3, 3.4, 1.24 and 0.85e-7
+// in 384^3.  The 81 gathers of a marker go through the cache hierarchy (the
+// markers of a home cell are adjacent, so a warp's gathers share lines) and are
+// what the kernel waits for: 271 us on 4 M markers in 512^3 at 64 registers, 300
+// at 80, against 38 us for the bytes; the home-relative sum took 282.
 template <typename R, typename FT>
 __global__ void __launch_bounds__(kGradThreads<R>, sizeof(R) == 4 ? 4 : 1)
     k_interp_gradient(Dims D, Grid<R> g, const R* __restrict__ x, const int32_t* __restrict__ home,
@@ -26,60 +81,86 @@ __global__ void __launch_bounds__(kGradThreads<R>, sizeof(R) == 4 ? 4 : 1)
   if (j >= M) return;
   const int64_t m = perm[j];
   const int32_t hc = home[j];
-  R out[3][3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int d = 0; d < 3; ++d) out[c][d] = R(0);
-  if (hc >= 0) {
+  bool ok = hc >= 0;
+  AxisEnds<R> f[3];
+  int xs[3], rows[3][3];
+  R z01[3], dz01[3], zm, dzm;   // along z the middle node too: E_0 + E_1 and its slope, E_0 and its slope
+  if (ok) {
     int i[3];
     decode_home(hc, D, i);
-    AxisForm<R, 4> f[3];
-    R d0[3][3], d1[3][3];
-    bool ok = true;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const AxisNodes<R> s = axis_nodes(g.ax[d], i[d], x[d * M + m]);
-      ok = axis_form<4>(s, inv_eps2, f[d]) && ok;
-      axis_slopes(s, f[d], inv_eps2, R(1) / s.w[1], d0[d], d1[d]);
-    }
-    if (ok) {
-      const int64_t N = (int64_t)D.n[0] * D.n[1] * D.n[2];
-      int xs[3], rows[3][3];
-      support_offsets(g, i, xs, rows);
-      const FT* uc[3] = {u, u + N, u + 2 * N};
-      R mid[3];
+      AxisForm<R, 4> a;
+      R d0[3], d1[3];
+      ok = axis_form<4>(s, inv_eps2, a) && ok;
+      axis_slopes(s, a, inv_eps2, R(1) / s.w[1], d0, d1);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) mid[c] = field_value<R, FT>(uc[c] + rows[1][1] + xs[1]);
+      for (int q = 0; q < 2; ++q) {
+        f[d].e0[q] = a.e0[2 * q];
+        f[d].e1[q] = a.e1[2 * q];
+        f[d].d0[q] = d0[2 * q];
+        f[d].d1[q] = d1[2 * q];
+      }
+      if (d == 2) {
+        zm = a.e0[1];
+        dzm = d0[1];
 #pragma unroll
-      for (int cz = 0; cz < 3; ++cz) {
-        const R z0 = f[2].e0[cz], z01 = z0 + f[2].e1[cz], dz0 = d0[2][cz], dz01 = dz0 + d1[2][cz];
-#pragma unroll
-        for (int cy = 0; cy < 3; ++cy) {
-          const R y0 = f[1].e0[cy], y1 = f[1].e1[cy], dy0 = d0[1][cy], dy1 = d1[1][cy];
-          const R k0 = y0 * z0, k1 = y0 * z01 + y1 * z0;
-          const R ky0 = dy0 * z0, ky1 = dy0 * z01 + dy1 * z0;
-          const R kz0 = y0 * dz0, kz1 = y0 * dz01 + y1 * dz0;
-#pragma unroll
-          for (int cx = 0; cx < 3; ++cx) {
-            const R e0 = f[0].e0[cx], e1 = f[0].e1[cx];
-            const R dphi[3] = {d0[0][cx] * k1 + d1[0][cx] * k0, e0 * ky1 + e1 * ky0, e0 * kz1 + e1 * kz0};
-            const int o = rows[cz][cy] + xs[cx];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const R v = field_value<R, FT>(uc[c] + o) - mid[c];
-#pragma unroll
-              for (int d = 0; d < 3; ++d) out[c][d] += dphi[d] * v;
-            }
-          }
+        for (int q = 0; q < 3; ++q) {
+          z01[q] = a.e0[q] + a.e1[q];
+          dz01[q] = d0[q] + d1[q];
         }
       }
     }
+    support_offsets(g, i, xs, rows);
   }
+  if (!ok) {
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
+    for (int q = 0; q < 9; ++q) G[q * M + m] = R(0);
+    return;
+  }
+  const int64_t N = (int64_t)D.n[0] * D.n[1] * D.n[2];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) G[(3 * c + d) * M + m] = out[c][d];
+  for (int c = 0; c < 3; ++c) {
+    const FT* uc = u + c * N;
+    R out[3] = {R(0), R(0), R(0)}, v_mid = R(0), w_mid = R(0);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const int cz = t == 0 ? 1 : t == 1 ? 0 : 2;   // the middle plane first: the others are taken against it
+      R v[3], e0[3], e1[3], d0[3], d1[3];           // per row: the middle node and the sums over x without it
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const FT* ur = uc + rows[cz][b];
+        v[b] = field_value<R, FT>(ur + xs[1]);
+        const R lo = field_value<R, FT>(ur + xs[0]) - v[b], hi = field_value<R, FT>(ur + xs[2]) - v[b];
+        e0[b] = ends(f[0].e0, lo, hi);
+        e1[b] = ends(f[0].e1, lo, hi);
+        d0[b] = ends(f[0].d0, lo, hi);
+        d1[b] = ends(f[0].d1, lo, hi);
+      }
+      const R e0l = (e0[0] - e0[1]) + (v[0] - v[1]), e0h = (e0[2] - e0[1]) + (v[2] - v[1]);
+      const R e1l = e1[0] - e1[1], e1h = e1[2] - e1[1];
+      const R d0l = d0[0] - d0[1], d0h = d0[2] - d0[1], d1l = d1[0] - d1[1], d1h = d1[2] - d1[1];
+      const AxisEnds<R>& y = f[1];
+      // Sums over the plane: the coefficient of E_0 + E_1 along z, and that of E_0.
+      const R x1 = d0[1] + ends(y.e0, d0l, d0h), x0 = d1[1] + ends(y.e0, d1l, d1h) + ends(y.e1, d0l, d0h);
+      const R y1 = ends(y.d0, e0l, e0h), y0 = ends(y.d0, e1l, e1h) + ends(y.d1, e0l, e0h);
+      const R w1 = e0[1] + ends(y.e0, e0l, e0h), w0 = e1[1] + ends(y.e0, e1l, e1h) + ends(y.e1, e0l, e0h);
+      const R z0 = cz == 1 ? zm : f[2].e0[cz / 2], dz0 = cz == 1 ? dzm : f[2].d0[cz / 2];
+      out[0] += z01[cz] * x1 + z0 * x0;
+      out[1] += z01[cz] * y1 + z0 * y0;
+      out[2] += dz0 * w0;
+      if (cz == 1) {
+        v_mid = v[1];
+        w_mid = w1;
+      } else {
+        out[2] += dz01[cz] * ((w1 - w_mid) + (v[1] - v_mid));
+      }
+    }
+    if (!isfinite(out[0] + out[1] + out[2])) plain_sum<R, FT>(f, uc, xs, rows, out);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) G[(3 * c + d) * M + m] = out[d];
+  }
 }
 
 template <typename R, typename FT>
