@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
                                                            const int32_t* __restrict__ n_items_p,
                                                            const int32_t* __restrict__ offsets,
                                                            const int32_t* __restrict__ counts, int64_t M, int64_t cap,
-                                                           const float* __restrict__ F, FT* __restrict__ f) {
+                                                           int max_bits, const float* __restrict__ F,
+                                                           FT* __restrict__ f) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NT = kSpreadThreads, CHUNK = kChunkPer * NT;
   const int ly = LY ? LY : tl.l[1], lz = LZ ? LZ : tl.l[2];   // compile-time when specialised
@@ -173,10 +174,12 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
     if (it + 1 < last) b = items[it + 1];       // the next tile's header, while this one is worked on
     unsigned next_start = start, next_end = end;
     for (unsigned j0 = start & ~3u; j0 < end; j0 += CHUNK) {
+      const unsigned stop = min(end, j0 + CHUNK);
+      const int bits = min(scale_bits(stop - max(start, j0)), max_bits);
       tag = tag == 255 ? 1 : tag + 1;
       float sum[3] = {0.f, 0.f, 0.f};
       const int n = list_runs<NT>(
-          home, start, end, j0, runs, s_cnt,
+          home, start, stop, j0, runs, s_cnt,
           [&](unsigned j, int at) {
             const int64_t m = perm[j];
             const float c = cl[j];
@@ -189,7 +192,7 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
           },
           [&] { publish_sums<NT>(sum, s_red); },
           [&] {
-            if (tid < 3) chunk_scale<NT>(s_red, tid, &s_scale);
+            if (tid < 3) chunk_scale<NT>(s_red, tid, bits, &s_scale);
           });
       if (it + 1 < last) {
         next_start = offsets[b];
@@ -203,13 +206,14 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
       o[1] &= ~((1 << ly) - 1);
       o[2] &= ~((1 << lz) - 1);
       if (kind == kFixed) {
+        const float limit = __uint_as_float((unsigned)(128 - bits) << 23);   // 2^(1 - bits)
         if (quad)
           add_runs<FT, true, NT, CHUNK>(D, o, n, runs, home, sv, j0, phi, cap, M, s_scale.inv, acc, A.AX, A.PS, A.ACC,
-                                        A.AY, tags, tag, f);
+                                        A.AY, tags, tag, limit, f);
         else
           add_runs<FT, false, NT, CHUNK>(D, o, n, runs, home, sv, j0, phi, cap, M, s_scale.inv, acc, A.AX, A.PS,
-                                         A.ACC, A.AY, tags, tag, f);
-        if (quad && it + 1 < last && j0 + CHUNK >= end)
+                                         A.ACC, A.AY, tags, tag, limit, f);
+        if (quad && it + 1 < last && stop == end)
           prefetch_tile(phi, home, perm, cl, cap, next_start, next_end);
         __syncthreads();
         flush_rows<FT, VEC, LX, NT>(D, o, A, acc, tags, tag, s_scale.unit, f);
@@ -365,8 +369,13 @@ static cudaError_t launch_spread_one(const mls_ctx* ctx, const mls_transfer* T, 
   const float* phi = (const float*)T->phi;
   const float* c = (const float*)T->c;
   int64_t M = T->M, cap = T->cap;
+  // Accumulating |phi| < 1/2 only (two scale bits) sends the node next to the
+  // marker past the accumulator where phi exceeds that: with the quadratic basis
+  // (0.61 at a cell centre, eps = 1), and with the linear one at
+  // (1 + 2 exp(-1/eps^2))^-3 > 1/2, eps < 0.7.  There one bit is the most.
+  int max_bits = ctx->opt.basis == 4 && ctx->opt.eps >= 0.75 ? 2 : 1;
   void* args[] = {&D, &tl, (void*)&phi, (void*)&c, (void*)&T->home, (void*)&T->perm, (void*)&T->items,
-                  (void*)&T->n_items, (void*)&T->offsets, (void*)&T->counts, &M, &cap, (void*)&F, &f};
+                  (void*)&T->n_items, (void*)&T->offsets, (void*)&T->counts, &M, &cap, &max_bits, (void*)&F, &f};
   return cudaLaunchKernel(spread_kernel<FT, VEC>(tl.l[0], tl.l[1], tl.l[2]), dim3(ctx->spread_grid), dim3(ctx->spread_threads), args,
                           spread_smem_bytes(ctx), s);
 }

@@ -48,6 +48,13 @@ __device__ __forceinline__ int tile_at(const int32_t* __restrict__ items, const 
   return lo;
 }
 
+// max(|a|, |b|, |c|), NaN if one is.
+__device__ __forceinline__ float max_abs(float a, float b, float c) {
+  float r;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // One node's term of a run in fixed point (the same bits wherever it is formed).
 __device__ __forceinline__ int run_term(float4 p, float4 v) {
   return __float2int_rn(__fmaf_rn(p.x, v.x, __fmaf_rn(p.y, v.y, __fmaf_rn(p.z, v.z, __fmul_rn(p.w, v.w)))));
@@ -67,12 +74,18 @@ __device__ __forceinline__ void publish_sums(float sum[3], float* red) {
   }
 }
 
-// Fixed-point scale of a chunk.  Terms with |phi| < 2 are accumulated, so no
-// cell's sum exceeds 2 S, S the chunk's sum of |c_l F_l| of that component
-// (rounded up by 1e-4, which covers its own rounding); with S < 2^ex the unit
-// 2^(ex - 30) keeps every sum inside 32 bits.  That is finer than a scale from
-// the largest term (unit 2^-22 of it or less) as soon as the mean |c_l F_l| is
-// below a quarter of the largest at 512 markers, or the chunk is smaller.
+// Fixed-point scale of a chunk.  Terms with |phi| < 2^(1 - e) are accumulated
+// (e = scale_bits), so no cell's sum exceeds 2^(1 - e) S, S the chunk's sum of
+// |c_l F_l| of that component (rounded up by 1e-4, which covers its own
+// rounding); with S < 2^ex the unit 2^(ex - 30 - e) keeps every sum inside 32
+// bits.  e grows with the chunk so that the unit is never coarser than 2^-22 of
+// the largest |c_l F_l|, which equal forces need: S is at most 2^(7 + e) times
+// the largest.  With e = 0 for all chunks a full chunk of equal forces had a unit
+// four times as coarse and an error of 2.4e-7 of f, against 0.74e-7 so (1 024 000
+// markers of 5 120-face bodies in 128^3); forces that differ have a finer unit,
+// the sum being smaller (noise: 1.9e-6, now 4.9e-7 there).  The launch caps e at 1
+// where phi itself exceeds 1/2.
+__device__ __forceinline__ int scale_bits(unsigned markers) { return markers <= 128 ? 0 : markers <= 256 ? 1 : 2; }
 enum ChunkScale { kZero, kFixed, kDirect };
 struct Scale {
   float unit[3], inv[3];
@@ -80,14 +93,14 @@ struct Scale {
 };
 // Component q of the scale, by one thread, from the warps' sums.
 template <int NT>
-__device__ __forceinline__ void chunk_scale(const float* red, int q, Scale* out) {
+__device__ __forceinline__ void chunk_scale(const float* red, int q, int bits, Scale* out) {
   float s = red[q];
   for (int w = 1; w < NT / 32; ++w) s += red[3 * w + q];
   out->kind[q] = s == 0.f ? kZero : kFixed;
   s *= 1.0001f;
   if (!isfinite(s)) out->kind[q] = kDirect;
   // The exponent field of s < 2^ex is ex + 126 (0 below the normal numbers).
-  const int sh = min(30 + 126 - (int)((__float_as_uint(s) >> 23) & 255u), 126);
+  const int sh = min(30 + bits + 126 - (int)((__float_as_uint(s) >> 23) & 255u), 126);
   out->inv[q] = __uint_as_float((unsigned)(127 + sh) << 23);
   out->unit[q] = __uint_as_float((unsigned)(127 - sh) << 23);
 }
@@ -121,13 +134,14 @@ __device__ __forceinline__ void add_direct(const Dims& D, const int i[3], const 
 // in the same instruction are serialised, so every third lane starts with
 // another component: only its pointers differ (wavefronts per atomic on a
 // model of the mixed bodies: 4.9 without, 2.9 with ACC = 8 or 20 mod 32).
-// Terms with some |phi| >= 2 or a NaN in their group of four go to f directly.
+// Terms with some |phi| >= limit (chunk_scale's 2^(1 - e)) or a NaN in their
+// group of four go to f directly.
 template <typename FT, bool QUAD, int NT, int CHUNK>
 __device__ __forceinline__ void add_runs(const Dims& D, const int o[3], int n, const int* runs,
                                          const int32_t* __restrict__ home,
                                          const float* sv, unsigned j0, const float* __restrict__ phi, int64_t cap,
                                          int64_t M, const float* scale, int* acc, int AX, int PS, int ACC, int AY,
-                                         unsigned char* tags, unsigned char tag, FT* __restrict__ f) {
+                                         unsigned char* tags, unsigned char tag, float limit, FT* __restrict__ f) {
   const int c0 = threadIdx.x % 3, c1 = c0 == 2 ? 0 : c0 + 1, c2 = c0 == 0 ? 2 : c0 - 1;
   const float s0 = scale[c0], s1 = scale[c1], s2 = scale[c2];
   for (int t = threadIdx.x; t < 3 * n; t += NT) {
@@ -156,28 +170,25 @@ __device__ __forceinline__ void add_runs(const Dims& D, const int o[3], int n, c
     int* a0 = acc + c0 * ACC + base;
     int* a1 = acc + c1 * ACC + base;
     int* a2 = acc + c2 * ACC + base;
-    unsigned bits = 0;
+    float most = 0.f;
 #pragma unroll
     for (int cy = 0; cy < 3; ++cy) {
       tags[z * AY + y + cy] = tag;
 #pragma unroll
       for (int cx = 0; cx < 3; ++cx) {
         const float4 pk = p[3 * cy + cx];
-        bits |= __float_as_uint(pk.x) | __float_as_uint(pk.y);
-        bits |= __float_as_uint(pk.z) | __float_as_uint(pk.w);
+        most = max_abs(max_abs(most, pk.x, pk.y), pk.z, pk.w);
         atomicAdd(a0 + cy * AX + cx, run_term(pk, v0));
         atomicAdd(a1 + cy * AX + cx, run_term(pk, v1));
         atomicAdd(a2 + cy * AX + cx, run_term(pk, v2));
       }
     }
-    // |p| < 2 <=> bit 30 is clear; otherwise what was added is taken back and
-    // the node's terms go to f.
-    if (bits & 0x40000000u) {
+    // What a node with a term out of the limit added is taken back, and its terms
+    // go to f.
+    if (!(most < limit)) {
       for (int k = 0; k < 9; ++k) {
         const float4 pk = phi_group<QUAD>(plane + k * cap, left);
-        if (((__float_as_uint(pk.x) | __float_as_uint(pk.y) | __float_as_uint(pk.z) | __float_as_uint(pk.w)) &
-             0x40000000u) == 0)
-          continue;
+        if (max_abs(max_abs(0.f, pk.x, pk.y), pk.z, pk.w) < limit) continue;
         const int at = k / 3 * AX + k % 3;
         atomicAdd(a0 + at, -run_term(pk, v0));
         atomicAdd(a1 + at, -run_term(pk, v1));
