@@ -270,7 +270,7 @@ constexpr int kQuad = 10;  // size of the quadratic basis (the linear one has 4)
 template <typename R, int MB>
 struct AxisForm {
   R e0[3], e1[3], e2[MB == 4 ? 1 : 3];
-  R m, v, g;      // mean and variance of xi under n, g = m / v
+  R m, v, iv, g;  // mean and variance of xi under n, 1 / v, g = m / v
   R c3, q2;    // quadratic: third central moment and sum_a n_a P2(xi_a)^2
 };
 
@@ -301,7 +301,8 @@ __device__ __forceinline__ bool axis_form(const AxisNodes<R>& s, R inv_eps2, Axi
   for (int a = 0; a < 3; ++a) nc[a] = f.e0[a] * c[a];
   f.v = nc[0] * c[0] + nc[1] * c[1] + nc[2] * c[2];
   f.m = mu - s.t;
-  f.g = f.m * recip(f.v);
+  f.iv = recip(f.v);
+  f.g = f.m * f.iv;
 #pragma unroll
   for (int a = 0; a < 3; ++a) f.e1[a] = -(nc[a] * f.g);
   if constexpr (MB != 4) {
@@ -338,7 +339,7 @@ __device__ __forceinline__ void axis_slopes(const AxisNodes<R>& s, const AxisFor
     nc[a] = f.e0[a] * c[a];
     c3 += nc[a] * c[a] * c[a];
   }
-  const R bh = beta * inv_h, dg = (beta - (R(1) + beta * f.g * c3) / f.v) * inv_h;
+  const R bh = beta * inv_h, dg = (beta - (R(1) + beta * f.g * c3) * f.iv) * inv_h;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     d0[a] = bh * nc[a];
