@@ -251,9 +251,10 @@ int mls_spread(mls_ctx* ctx, const mls_transfer* T, const void* F, void* f, void
 /* One direct-forcing transfer (text after Eq. 6, then Eq. 7): interpolate
  * U_l = sum_k phi_k^l u_k, form the IBM force F_l = (V_b,l - U_l) / dt that
  * drives the fluid velocity at marker l to the desired V_b,l, and spread
- * f_k += sum_l c_l phi_k^l F_l.  In single-precision contexts the
- * interpolation kernel forms F as it stores U, and the spreading kernel
- * follows; double-precision contexts compose the separate kernels.
+ * f_k += sum_l c_l phi_k^l F_l.  In single-precision contexts this is one
+ * pass over the spreading tiles that reads phi once; a context whose tile does
+ * not fit one block's shared memory twice, a call whose u and f overlap, and
+ * double-precision contexts compose the separate kernels.
  *   u   device, field[3][nz][ny][nx]         Vb  device, real[3][M] desired velocity
  *   dt  time step (> 0)                      U   device, real[3][M] or NULL (not written)
  *   F   device, real[3][M] output forces     f   device, field[3][nz][ny][nx], accumulated

@@ -52,56 +52,6 @@ __global__ void __launch_bounds__(kBlock) k_interp(Dims D, const R* __restrict__
   U[2 * M + m] = s2;
 }
 
-// U_l = sum_k phi_k^l u_k (text after Eq. 6), single precision, with F also the
-// direct forcing F = (V_b - U) / dt: a block lists the runs of
-// kChunkPer * kInterpThreads stored markers and a thread per run gathers the
-// run's velocities through the cache hierarchy.  Dropped markers get U = F = 0.
-// What it cannot do without is phi once (108 bytes a marker); it waits for the
-// gathers, so warps count: 4 M markers in 512^3 take 173 us at 64 registers,
-// 182 at 80 (79 us for the bytes), 32 M in 1024^3 1.22 ms.  A brick of the
-// tile's field rows staged in shared memory and gathered marker by marker,
-// which this replaced, took 263 us and 1.55 ms: three loads per marker and node
-// instead of per run, and a barrier per tile on either side of the copy.
-template <typename FT, bool FORCE>
-__global__ void __launch_bounds__(kInterpThreads, 8) k_interp_runs(Dims D, const float* __restrict__ phi,
-                                                                   const int32_t* __restrict__ home,
-                                                                   const int32_t* __restrict__ perm, int64_t M,
-                                                                   int64_t cap, InterpOut<float, FT> io) {
-  constexpr int NT = kInterpThreads, CHUNK = kChunkPer * NT;
-  __shared__ int runs[CHUNK];
-  __shared__ int s_cnt[kChunkPer * (NT / 32)];
-  const unsigned j0 = blockIdx.x * (unsigned)CHUNK, end = (unsigned)min((int64_t)j0 + CHUNK, M);
-  const int n = list_runs<NT>(home, j0, end, j0, runs, s_cnt, [](unsigned, int) {}, [] {}, [] {});
-  for (int t = threadIdx.x; t < n; t += NT) {
-    const Run r(runs[t]);
-    const int64_t g = j0 + (r.first & ~3);
-    const int in = r.first & 3;
-    const int32_t h = home[j0 + r.first];
-    if (h < 0) {
-      for (int k = in; k < in + r.len; ++k) io.store_zero(perm[g + k], M);
-      continue;
-    }
-    int i[3];
-    decode_home(h, D, i);
-    float4 U[3];
-    if ((cap & 3) == 0)
-      gather_run<FT, true>(D, i, io.u, phi + g, cap, M - g, U);
-    else
-      gather_run<FT, false>(D, i, io.u, phi + g, cap, M - g, U);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (k >= in && k < in + r.len) {
-        const int64_t m = perm[g + k];
-        if constexpr (FORCE) {
-          io.store(m, M, at(U[0], k), at(U[1], k), at(U[2], k));
-        } else {
-#pragma unroll
-          for (int q = 0; q < 3; ++q) io.U[q * M + m] = at(U[q], k);
-        }
-      }
-  }
-}
-
 // f_k += sum_l c_l phi_k^l F_l (text after Eq. 7), single precision.
 // Persistent blocks walk the list of non-empty spreading tiles, taking up to
 // 512 markers of a tile at a time: a thread per marker forms c_l F_l and the
@@ -145,9 +95,7 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
   for (int r = tid; r < A.AY * A.AZ; r += NT) tags[r] = 0;
 
   // Every block takes tiles of about equal total weight, neighbours in the list;
-  // with fewer tiles than blocks, a share (whole groups of 32 markers) of one,
-  // since a small workload's time is that of a tile's chain from load to flush (a
-  // small box whose step took 25 us and 35 with whole tiles; others 87 -> 69).
+  // with fewer tiles than blocks, a share of one.
   if (n_items == 0) return;
   __shared__ int s_range[2];
   const int parts = min((int)gridDim.x / n_items, 8);
@@ -164,22 +112,15 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
   const int last = s_range[1];
   int b = it < last ? items[it] : 0;
   unsigned start = offsets[b], end = start + counts[b];
-  if (parts > 1) {
-    const unsigned first = start & ~3u, share = ((end - first + parts - 1) / parts + 31u) & ~31u;
-    const unsigned from = first + blockIdx.x % parts * share;
-    start = max(start, from);
-    end = min(end, from + share);
-  }
+  if (parts > 1) tile_part(blockIdx.x % parts, parts, start, end);
   for (; it < last; ++it) {
     if (it + 1 < last) b = items[it + 1];       // the next tile's header, while this one is worked on
     unsigned next_start = start, next_end = end;
     for (unsigned j0 = start & ~3u; j0 < end; j0 += CHUNK) {
-      const unsigned stop = min(end, j0 + CHUNK);
-      const int bits = min(scale_bits(stop - max(start, j0)), max_bits);
       tag = tag == 255 ? 1 : tag + 1;
       float sum[3] = {0.f, 0.f, 0.f};
       const int n = list_runs<NT>(
-          home, start, stop, j0, runs, s_cnt,
+          home, start, end, j0, runs, s_cnt,
           [&](unsigned j, int at) {
             const int64_t m = perm[j];
             const float c = cl[j];
@@ -192,7 +133,7 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
           },
           [&] { publish_sums<NT>(sum, s_red); },
           [&] {
-            if (tid < 3) chunk_scale<NT>(s_red, tid, bits, &s_scale);
+            if (tid < 3) chunk_scale<NT>(s_red, tid, min(scale_bits(min(end, j0 + CHUNK) - max(start, j0)), max_bits), &s_scale);
           });
       if (it + 1 < last) {
         next_start = offsets[b];
@@ -206,14 +147,13 @@ __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, 
       o[1] &= ~((1 << ly) - 1);
       o[2] &= ~((1 << lz) - 1);
       if (kind == kFixed) {
-        const float limit = __uint_as_float((unsigned)(128 - bits) << 23);   // 2^(1 - bits)
         if (quad)
-          add_runs<FT, true, NT, CHUNK>(D, o, n, runs, home, sv, j0, phi, cap, M, s_scale.inv, acc, A.AX, A.PS, A.ACC,
-                                        A.AY, tags, tag, limit, f);
+          add_runs<FT, true, NT, CHUNK>(D, o, n, runs, home, sv, j0, phi, cap, M, s_scale, acc, A.AX, A.PS, A.ACC,
+                                        A.AY, tags, tag, f);
         else
-          add_runs<FT, false, NT, CHUNK>(D, o, n, runs, home, sv, j0, phi, cap, M, s_scale.inv, acc, A.AX, A.PS,
-                                         A.ACC, A.AY, tags, tag, limit, f);
-        if (quad && it + 1 < last && stop == end)
+          add_runs<FT, false, NT, CHUNK>(D, o, n, runs, home, sv, j0, phi, cap, M, s_scale, acc, A.AX, A.PS,
+                                         A.ACC, A.AY, tags, tag, f);
+        if (quad && it + 1 < last && j0 + CHUNK >= end)
           prefetch_tile(phi, home, perm, cl, cap, next_start, next_end);
         __syncthreads();
         flush_rows<FT, VEC, LX, NT>(D, o, A, acc, tags, tag, s_scale.unit, f);
@@ -336,28 +276,13 @@ cudaError_t spread_configure(mls_ctx* ctx) {
   return configure_kernel(ctx, bf ? spread_kernel<__nv_bfloat16, false>(lx, ly, lz) : spread_kernel<float, false>(lx, ly, lz), smem);
 }
 
-template <typename FT>
-static void launch_interp_runs(const mls_ctx* ctx, const mls_transfer* T, const void* u, void* U, const void* Vb,
-                               double dt, void* F, cudaStream_t s) {
-  constexpr int64_t chunk = kChunkPer * kInterpThreads;
-  const int64_t N = (int64_t)ctx->n[0] * ctx->n[1] * ctx->n[2];
-  const InterpOut<float, FT> io{(const FT*)u, (float*)U, N, (const float*)Vb, F ? (float)(1.0 / dt) : 0.f, (float*)F};
-  auto kern = F ? k_interp_runs<FT, true> : k_interp_runs<FT, false>;
-  kern<<<(unsigned)((T->M + chunk - 1) / chunk), kInterpThreads, 0, s>>>(dims_of(ctx), (const float*)T->phi, T->home,
-                                                                        T->perm, T->M, T->cap, io);
-}
-
 cudaError_t launch_interp(const mls_ctx* ctx, const mls_transfer* T, const void* u, void* U, cudaStream_t s,
                           const void* Vb, double dt, void* F) {
   if (T->M == 0) return cudaSuccess;
+  if (ctx->opt.real != MLS_F64) return launch_tiles(ctx, T, u, Vb, dt, U, F, nullptr, s);
   const unsigned nt = block_threads(T->M, kBlock);
-  if (ctx->opt.real == MLS_F64)
-    k_interp<double, double><<<blocks_for(T->M, nt), nt, 0, s>>>(
-        dims_of(ctx), (const double*)T->phi, T->home, T->perm, T->M, T->cap, (const double*)u, (double*)U);
-  else if (ctx->opt.field == MLS_BF16)
-    launch_interp_runs<__nv_bfloat16>(ctx, T, u, U, Vb, dt, F, s);
-  else
-    launch_interp_runs<float>(ctx, T, u, U, Vb, dt, F, s);
+  k_interp<double, double><<<blocks_for(T->M, nt), nt, 0, s>>>(dims_of(ctx), (const double*)T->phi, T->home, T->perm,
+                                                               T->M, T->cap, (const double*)u, (double*)U);
   return cudaGetLastError();
 }
 

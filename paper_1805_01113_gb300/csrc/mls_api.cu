@@ -285,6 +285,7 @@ int mls_create(const mls_grid* grid, const mls_options* opt_in, mls_ctx** out) {
     return invalid("mls_create: spreading tile too large for shared memory; lower brick_log2");
   }
   cudaError_t e = spread_configure(c);
+  if (e == cudaSuccess) e = tiles_configure(c);
   if (e == cudaSuccess) e = collision_configure(c);
   if (e == cudaSuccess) e = sort_configure(c);
   if (e == cudaSuccess) e = mlp_configure();
