@@ -7,40 +7,36 @@
 
 namespace mls {
 
-// A group of threads (a warp where the cell states of a tile are small, else a
-// block) walks the non-empty tiles.  For a tile: zero the state of its
-// 2^(lx+ly+lz) home cells; every marker with a body index b > 0 claims its cell
+// Groups of threads (warps or whole blocks) walk the non-empty tiles.  For a
+// tile: zero the state of its 2^(lx+ly+lz) home cells; every marker with a body index b > 0 claims its cell
 // with compare-and-swap (0 -> b) and, finding another index there, sets the
 // cell to -1; then every marker reads its cell: -1 flags it.  The occupied
 // cells are written to `coll` when requested.  The final state of a cell does
 // not depend on the order of the updates (an empty cell takes the first index,
 // any second index makes it -1, and -1 is never overwritten).
+// Returns the colliding markers that the thread found.
 // Bound by the chain of dependent loads of a tile (its header, the order, the
-// body indices): a warp per tile keeps four times as many tiles in flight as a
-// block per tile and needs no block barriers, the markers of a tile of up to
-// 128 are loaded once, and the next tile's header is loaded ahead.  On 5.1 M
-// markers in 384^3, with the clearing of the cell array, 126 -> 108 us.
+// body indices); the markers of a tile of up to four per thread are loaded once,
+// and the next tile's header is loaded ahead.
 template <bool WARP>
-__global__ void __launch_bounds__(kSpreadThreads) k_collisions(Dims D, Tiles tl, const int32_t* __restrict__ home,
-                                                               const int32_t* __restrict__ perm,
-                                                               const int32_t* __restrict__ items,
-                                                               const int32_t* __restrict__ n_items_p,
-                                                               const int32_t* __restrict__ offsets,
-                                                               const int32_t* __restrict__ counts, int64_t M,
-                                                               const int32_t* __restrict__ body,
-                                                               int32_t* __restrict__ flag, int32_t* __restrict__ coll,
-                                                               unsigned long long* __restrict__ n_colliding) {
+__device__ __forceinline__ unsigned long long collide_tiles(const Dims& D, const Tiles& tl,
+                                                            const int32_t* __restrict__ home,
+                                                            const int32_t* __restrict__ perm,
+                                                            const int32_t* __restrict__ items, int n_items,
+                                                            const int32_t* __restrict__ offsets,
+                                                            const int32_t* __restrict__ counts,
+                                                            const int32_t* __restrict__ body,
+                                                            int32_t* __restrict__ flag, int32_t* __restrict__ coll) {
   extern __shared__ __align__(16) int state_all[];
   constexpr int G = WARP ? 32 : kSpreadThreads, PER = 4, GROUPS = kSpreadThreads / G;
   const int lx = tl.l[0], ly = tl.l[1], lz = tl.l[2];
   const int TC = 1 << (lx + ly + lz);
-  const int tid = threadIdx.x % G, lane = threadIdx.x & 31, group = threadIdx.x / G;
+  const int tid = threadIdx.x % G, group = threadIdx.x / G;
   int* state = state_all + group * TC;
   auto sync = [] {
     if (WARP) __syncwarp();
     else __syncthreads();
   };
-  const int n_items = *n_items_p;
   const int stride = gridDim.x * GROUPS;
   unsigned long long found = 0;
   int it = blockIdx.x * GROUPS + group;
@@ -122,8 +118,36 @@ __global__ void __launch_bounds__(kSpreadThreads) k_collisions(Dims D, Tiles tl,
     start = next_start;
     n = next_n;
   }
-  // Markers without support: never flagged.
+  return found;
+}
+
+// A warp per tile keeps four times as many tiles in flight as a block per tile
+// and needs no block barriers: 5.1 M markers in 384^3, with the clearing of the
+// cell array, 126 -> 108 us.  Where the tiles do not fill the device with blocks,
+// or twice over while they hold fewer than 512 markers on average, a tile's own
+// chain is what takes time and a block walks it sooner: 1.4 M markers of a dense
+// packing in 64^3 21 against 51 us, 16 000 markers in 48^3 3.4 against 5.8; 11.2 M
+// on 4 096 tiles in 128^3 take 129 by warps and 157 by blocks.
+// SMALL: the states of a block's four warps fit (tiles of up to 2^10 cells).
+template <bool SMALL>
+__global__ void __launch_bounds__(kSpreadThreads) k_collisions(Dims D, Tiles tl, const int32_t* __restrict__ home,
+                                                               const int32_t* __restrict__ perm,
+                                                               const int32_t* __restrict__ items,
+                                                               const int32_t* __restrict__ n_items_p,
+                                                               const int32_t* __restrict__ offsets,
+                                                               const int32_t* __restrict__ counts, int64_t M,
+                                                               const int32_t* __restrict__ body,
+                                                               int32_t* __restrict__ flag, int32_t* __restrict__ coll,
+                                                               unsigned long long* __restrict__ n_colliding) {
+  const int n_items = *n_items_p, lane = threadIdx.x & 31;
   const int64_t d0 = offsets[tl.nbins - 1];
+  const int blocks = gridDim.x;
+  unsigned long long found;
+  if (!SMALL || n_items < blocks || (n_items < 2 * blocks && d0 < 512 * (int64_t)n_items))
+    found = collide_tiles<false>(D, tl, home, perm, items, n_items, offsets, counts, body, flag, coll);
+  else
+    found = collide_tiles<true>(D, tl, home, perm, items, n_items, offsets, counts, body, flag, coll);
+  // Markers without support: never flagged.
   for (int64_t j = d0 + (int64_t)blockIdx.x * kSpreadThreads + threadIdx.x; j < M;
        j += (int64_t)gridDim.x * kSpreadThreads)
     flag[perm[j]] = 0;
@@ -134,20 +158,20 @@ __global__ void __launch_bounds__(kSpreadThreads) k_collisions(Dims D, Tiles tl,
   }
 }
 
-// A warp per tile while four tiles' states fit the default 48 KB of a block
-// several times over (2^10 cells: 16 KB, 14 blocks per SM); beyond, a block.
-static bool collide_by_warp(const mls_ctx* ctx) {
+// Four tiles' states fit the default 48 KB of a block several times over (2^10
+// cells: 16 KB, 14 blocks per SM).
+static bool collide_small(const mls_ctx* ctx) {
   return ctx->tiles.l[0] + ctx->tiles.l[1] + ctx->tiles.l[2] <= 10;
 }
 static size_t collide_smem(const mls_ctx* ctx) {
   const int* l = ctx->tiles.l;
-  return ((size_t)4 << (l[0] + l[1] + l[2])) * (collide_by_warp(ctx) ? kSpreadThreads / 32 : 1);
+  return ((size_t)4 << (l[0] + l[1] + l[2])) * (collide_small(ctx) ? kSpreadThreads / 32 : 1);
 }
 
 cudaError_t launch_collisions(const mls_ctx* ctx, const mls_transfer* T, const int32_t* body, int32_t* flag,
                               int32_t* coll, unsigned long long* n_colliding, cudaStream_t s) {
   if (T->M == 0) return cudaSuccess;
-  auto kern = collide_by_warp(ctx) ? k_collisions<true> : k_collisions<false>;
+  auto kern = collide_small(ctx) ? k_collisions<true> : k_collisions<false>;
   kern<<<ctx->collision_grid, kSpreadThreads, collide_smem(ctx), s>>>(dims_of(ctx), ctx->tiles, T->home, T->perm,
                                                                       T->items, T->n_items, T->offsets, T->counts,
                                                                       T->M, body, flag, coll, n_colliding);
@@ -155,7 +179,7 @@ cudaError_t launch_collisions(const mls_ctx* ctx, const mls_transfer* T, const i
 }
 
 cudaError_t collision_configure(mls_ctx* ctx) {
-  auto kern = collide_by_warp(ctx) ? k_collisions<true> : k_collisions<false>;
+  auto kern = collide_small(ctx) ? k_collisions<true> : k_collisions<false>;
   const int smem = (int)collide_smem(ctx);
   cudaError_t e;
   if ((e = raise_smem_limit((const void*)kern, smem)) != cudaSuccess) return e;
