@@ -343,7 +343,8 @@ int mls_transfer_status(const mls_transfer* T, void* stream, mls_status* out);
  * s = (s_z*n + s_y)*n + s_x, class = home index along the one non-uniform
  * axis (0 when all are uniform); a row holds the 27 exact shape-function
  * values of the sub-node (k = 9 c + 3 b + a) and one zero pad, so rows are
- * 16-byte aligned. */
+ * 16-byte aligned.  MLS_FAST builds do not need it: they read per-axis factors
+ * of these functions, a few hundred bytes per class, made on the first build. */
 #define MLS_TABLE_ROW 28
 int mls_fast_table(mls_ctx* ctx, void* stream, const void** table, int64_t* n_classes, int32_t* n_sub);
 
@@ -361,8 +362,9 @@ int mls_fast_table(mls_ctx* ctx, void* stream, const void** table, int64_t* n_cl
  *     the library holds until the process exits;
  *   - limits: M <= MLS_NOALLOC_MAX_MARKERS and the context's spreading-tile
  *     count + 1 <= MLS_NOALLOC_MAX_BINS, else MLS_ERR_CAPACITY;
- *   - MLS_FAST needs the context's fast-MLS table to exist already (build it
- *     at set-up with mls_fast_table, which allocates), else MLS_ERR_UNSUPPORTED;
+ *   - MLS_FAST needs the context's fast-MLS factors to exist already (an
+ *     MLS_FAST build of mls_build_transfer, mls_fast_table or mls_load of a
+ *     table makes them at set-up, with an allocation), else MLS_ERR_UNSUPPORTED;
  *   - MLS_SURROGATE is not offered (its exact-MLS fallback and network
  *     buffers are not part of the static array): MLS_ERR_UNSUPPORTED;
  *   - no counters are returned: dropped markers are those with home = -1.
@@ -438,20 +440,24 @@ int mls_surrogate_loss_grad(mls_ctx* ctx, const float* X, const float* T, int32_
 /* ---- checkpoint / resume ------------------------------------------------
  * The context's marker-independent state: the fast-MLS table (Section 2,
  * Fig. 1b/1c; real[n_classes][n_sub^3][27] shape functions at the sub-Eulerian
- * points) when an MLS_FAST build or mls_fast_table has made it, and the
- * surrogate's float32 parameters when trained or set.  The file holds a
+ * points) when the context has built with MLS_FAST or mls_fast_table has made
+ * it, and the surrogate's float32 parameters when trained or set.  The per-axis
+ * factors that MLS_FAST builds read are not stored: they follow from what the
+ * key covers, and mls_load makes them with the table.  The file holds a
  * versioned header, a 64-bit key over the grid (n, periodic, every face), eps,
  * n_sub, the basis size and the real precision, the present blocks, and a
  * trailing checksum.
  *
  * mls_save: synchronises the device, writes `path` (host file name) through a
  * temporary "<path>.partial" that is renamed into place.  A context with
- * neither block writes a header-only file.  MLS_ERR_INVALID_ARG when the file
- * cannot be written; CUDA errors as MLS_ERR_CUDA.
+ * neither block writes a header-only file; one that has built with MLS_FAST but
+ * has no table yet makes it first (an allocation).  MLS_ERR_INVALID_ARG when the
+ * file cannot be written; CUDA errors as MLS_ERR_CUDA.
  *
  * mls_load: reads and validates the whole file before changing the context;
- * then allocates the table if absent, copies it in (after a device
- * synchronise, so launches still using the old table finish first), and sets
+ * then allocates the table (and makes the builds' factors) if absent, copies
+ * it in (after a device synchronise, so launches still using the old table
+ * finish first), and sets
  * the surrogate parameters as mls_surrogate_params(set = 1) does.  An
  * existing table is overwritten in place: its device address, and so any
  * CUDA graph captured with it, stays valid.

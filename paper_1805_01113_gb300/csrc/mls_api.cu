@@ -121,11 +121,41 @@ int64_t fast_axis_offsets(const mls_ctx* ctx, int64_t at[3]) {
   return n;
 }
 
-size_t fast_axes_begin(const mls_ctx* ctx) { return (fast_table_bytes(ctx) + 255) & ~(size_t)255; }
-
-size_t fast_alloc_bytes(const mls_ctx* ctx) {
+size_t fast_axes_bytes(const mls_ctx* ctx) {
   int64_t at[3];
-  return fast_axes_begin(ctx) + (size_t)fast_axis_offsets(ctx, at) * (ctx->opt.real == MLS_F64 ? 8 : 4);
+  return (size_t)fast_axis_offsets(ctx, at) * (ctx->opt.real == MLS_F64 ? 8 : 4);
+}
+
+// One of the context's two fast-MLS arrays: allocated, filled and waited for.
+static int make_fast(mls_ctx* ctx, void** array, size_t bytes, cudaError_t (*launch)(mls_ctx*, cudaStream_t),
+                     const char* name, cudaStream_t s) {
+  if (*array) return MLS_OK;
+  cudaError_t e = cudaMalloc(array, bytes);
+  if (e != cudaSuccess) {
+    *array = nullptr;
+    return cuda_fail(e, "fast-MLS table allocation");
+  }
+  const int slot = timer_begin(ctx, name, s);
+  e = launch(ctx, s);
+  timer_end(ctx, slot, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
+    cudaFree(*array);
+    *array = nullptr;
+    return cuda_fail(e, "fast-MLS table build");
+  }
+  return MLS_OK;
+}
+
+int ensure_fast_axes(mls_ctx* ctx, cudaStream_t s) {
+  if (ctx->fast_axes) return MLS_OK;
+  const int rc = fast_table_layout(ctx);
+  return rc != MLS_OK ? rc : make_fast(ctx, &ctx->fast_axes, fast_axes_bytes(ctx), launch_fast_axes, "fast_axes", s);
+}
+
+int ensure_fast_table(mls_ctx* ctx, cudaStream_t s) {
+  const int rc = ensure_fast_axes(ctx, s);
+  return rc != MLS_OK ? rc : make_fast(ctx, &ctx->table, fast_table_bytes(ctx), launch_fast_table, "fast_table", s);
 }
 
 }  // namespace mls
@@ -171,6 +201,7 @@ static void free_ctx(mls_ctx* c) {
     cudaFree(c->widths_f[d]);
   }
   cudaFree(c->table);
+  cudaFree(c->fast_axes);
   cudaFree(c->mlp_theta);
   cudaFree(c->mlp_pack);
   cudaFree(c->refine_ws);
@@ -214,6 +245,7 @@ int mls_create(const mls_grid* grid, const mls_options* opt_in, mls_ctx** out) {
   if (!c) return invalid("mls_create: out of host memory");
   c->opt = opt;
   c->table = nullptr;
+  c->fast_axes = nullptr;
   c->refine_ws = nullptr;
   c->refine_ws_bytes = 0;
   c->n_classes = 0;
@@ -462,28 +494,6 @@ int mls_refine_markers(mls_ctx* ctx, const void* vertices, int64_t n_vertices, c
   return MLS_OK;
 }
 
-static int ensure_table(mls_ctx* ctx, cudaStream_t s) {
-  if (ctx->table) return MLS_OK;
-  int rc = fast_table_layout(ctx);
-  if (rc != MLS_OK) return rc;
-  cudaError_t e = cudaMalloc(&ctx->table, fast_alloc_bytes(ctx));
-  if (e != cudaSuccess) {
-    ctx->table = nullptr;
-    return cuda_fail(e, "fast-MLS table allocation");
-  }
-  const int slot = timer_begin(ctx, "fast_table", s);
-  e = launch_fast_table(ctx, s);
-  if (e == cudaSuccess) e = launch_fast_axes(ctx, s);
-  timer_end(ctx, slot, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
-    cudaFree(ctx->table);
-    ctx->table = nullptr;
-    return cuda_fail(e, "fast-MLS table build");
-  }
-  return MLS_OK;
-}
-
 // The build of mls_build_transfer; with u (and U) also the interpolation of
 // mls_interpolate, fused into the exact linear-basis build kernel.
 static int build_impl(mls_ctx* ctx, mls_transfer* T, const void* x, const void* area, int64_t M, int32_t method,
@@ -506,7 +516,7 @@ static int build_impl(mls_ctx* ctx, mls_transfer* T, const void* x, const void* 
   if (M > 0 && (!x || !area)) return invalid("mls_build_transfer: NULL marker arrays");
   cudaStream_t s = (cudaStream_t)stream;
   if (method == MLS_FAST) {
-    int rc = ensure_table(ctx, s);
+    int rc = ensure_fast_axes(ctx, s);
     if (rc != MLS_OK) return rc;
   }
   T->M = M;
@@ -694,7 +704,7 @@ int mls_transfer_status(const mls_transfer* T, void* stream, mls_status* out) {
 
 int mls_fast_table(mls_ctx* ctx, void* stream, const void** table, int64_t* n_classes, int32_t* n_sub) {
   if (!ctx || !table || !n_classes || !n_sub) return invalid("mls_fast_table: NULL argument");
-  int rc = ensure_table(ctx, (cudaStream_t)stream);
+  int rc = ensure_fast_table(ctx, (cudaStream_t)stream);
   if (rc != MLS_OK) return rc;
   *table = ctx->table;
   *n_classes = ctx->n_classes;

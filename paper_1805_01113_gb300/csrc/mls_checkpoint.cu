@@ -92,6 +92,11 @@ int mls_save(mls_ctx* ctx, const char* path) {
   // Tables and parameters are written by earlier launches on any stream.
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(e, "mls_save");
+  // A context that has built with MLS_FAST saves its table, which those builds do not make.
+  if (ctx->fast_axes) {
+    const int rc = ensure_fast_table(ctx, nullptr);
+    if (rc != MLS_OK) return rc;
+  }
   Writer w;
   w.add(kMagic, sizeof(kMagic));
   w.put<uint32_t>(kVersion);
@@ -205,18 +210,19 @@ int mls_load(mls_ctx* ctx, const char* path) {
 
   cudaError_t e;
   if (table_data) {
+    // The builds' factors follow from what the key covers; the table is the file's.
+    const int rc = ensure_fast_axes(ctx, nullptr);
+    if (rc != MLS_OK) return rc;
     const bool fresh = !ctx->table;
-    if (fresh && (e = cudaMalloc(&ctx->table, fast_alloc_bytes(ctx))) != cudaSuccess) {
+    if (fresh && (e = cudaMalloc(&ctx->table, table_bytes)) != cudaSuccess) {
       ctx->table = nullptr;
       return cuda_fail(e, "mls_load: table allocation");
     }
     // A table in use by launches still in flight is replaced only after they end.
     if ((e = cudaDeviceSynchronize()) != cudaSuccess ||
-        (e = cudaMemcpy(ctx->table, table_data, table_bytes, cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (fresh && ((e = launch_fast_axes(ctx, nullptr)) != cudaSuccess ||
-                   (e = cudaStreamSynchronize(nullptr)) != cudaSuccess))) {
-      // A table allocated here never holds partial contents: later fast builds
-      // rebuild it instead.
+        (e = cudaMemcpy(ctx->table, table_data, table_bytes, cudaMemcpyHostToDevice)) != cudaSuccess) {
+      // A table allocated here never holds partial contents: a later
+      // mls_fast_table builds it instead.
       if (fresh) {
         cudaFree(ctx->table);
         ctx->table = nullptr;

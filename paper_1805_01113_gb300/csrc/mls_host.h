@@ -37,9 +37,10 @@ struct mls_ctx {
   int nbk[3];
   std::vector<double> faces_host[3];
   mls::Tiles tiles;
-  // Fast-MLS table, real[n_classes][n_sub^3][kTableRow], then (from
-  // fast_axes_begin) the per-axis factors the builds read; class axis -1 when uniform.
+  // Fast-MLS: the table, real[n_classes][n_sub^3][kTableRow] (mls_fast_table and
+  // checkpoints), and the per-axis factors the builds read; class axis -1 when uniform.
   void* table;
+  void* fast_axes;
   int64_t n_classes;
   int class_axis;
   // Persistent grid of the spreading kernel (blocks resident on the device).
@@ -132,11 +133,13 @@ int fast_table_layout(mls_ctx* ctx);
 size_t fast_table_bytes(const mls_ctx* ctx);
 // The per-axis factors of the table: values per sub-node (E_0, E_1 and, for
 // the quadratic basis, E_2 at three nodes, padded to 16-byte rows), where each
-// axis starts, where they start behind the table, and the bytes of both.
+// axis starts, and the bytes of all three.
 __host__ __device__ constexpr int fast_row(int basis) { return basis == 4 ? 8 : 12; }
 int64_t fast_axis_offsets(const mls_ctx* ctx, int64_t at[3]);
-size_t fast_axes_begin(const mls_ctx* ctx);
-size_t fast_alloc_bytes(const mls_ctx* ctx);
+size_t fast_axes_bytes(const mls_ctx* ctx);
+// Make the factors, or the table and the factors, unless they exist.
+int ensure_fast_axes(mls_ctx* ctx, cudaStream_t s);
+int ensure_fast_table(mls_ctx* ctx, cudaStream_t s);
 
 // Phase helpers: every call opens and closes an NVTX range named after the
 // phase; CUDA events are recorded only when ctx->timing is on.

@@ -83,7 +83,7 @@ extern "C" int mls_build_transfer_noalloc(mls_ctx* ctx, const void* x, const voi
     return fail(MLS_ERR_INVALID_ARG, "mls_build_transfer_noalloc: NULL array");
   if (ld_phi < M || ld_phi > 0x7fffffffLL - 1)
     return fail(MLS_ERR_INVALID_ARG, "mls_build_transfer_noalloc: ld_phi must be in [M, 2^31-2]");
-  if (method == MLS_FAST && !ctx->table)
+  if (method == MLS_FAST && !ctx->fast_axes)
     return fail(MLS_ERR_UNSUPPORTED,
                 "mls_build_transfer_noalloc: the fast-MLS table does not exist yet; call mls_fast_table first");
   int dev = -1;
