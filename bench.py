@@ -840,11 +840,8 @@ def run_ours(a, rank, world, local):
                                         "U": _errs(ob["U"], ref["U"]), "f": _errs(ob["f"], ref["fv"]),
                                         "bound_stated": 1e-2,
                                         "kernels_ms": {k: round(v[1] / v[0], 5) for k, v in kb.items() if v[0]}}
-            c0 = api.Context(w.faces, w.periodic, real="f32", refine=0, brick_log2=tiles)
-            o0 = sample_outputs(c0, "exact", torch.float32)
-            precision["f32_solve_no_refinement"] = {"phi": _errs(o0["phi"], ref["phi"])}
-            precision["f32_solve_one_refinement"] = {"phi": errs["exact"]["phi_vs_exact"],
-                                                     "fp64_fallbacks": ctx.status(T)["refined_fp64"]}
+            precision["f32_shape_functions"] = {"phi": errs["exact"]["phi_vs_exact"],
+                                                "fp64_fallbacks": ctx.status(T)["refined_fp64"]}
         if "surrogate" in others:
             # The surrogate's gate (linear-reproduction residual of the raw network
             # output) at several thresholds: fallback rate and build time on the

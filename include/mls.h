@@ -84,7 +84,8 @@ typedef struct {
   int32_t n_sub;         /* fast-MLS sub-Eulerian points per axis (Fig. 1b/1c), 3..33, default 9 */
   int32_t brick_log2[3]; /* spreading tile of 2^b home cells per axis, 1..5 each, default 3 */
   double cond_max;       /* MLS_F32 only: re-solve Eq. 6 in double when cond_1(A) exceeds this; <= 0 disables; default 1e6 */
-  int32_t refine;        /* MLS_F32 only: iterative-refinement steps of the solve, 0..2, default 1 */
+  int32_t refine;        /* 0..2, default 1; checked and otherwise without effect: the shape functions
+                            come in closed form, with no solve to refine */
   double residual_max;   /* MLS_SURROGATE: linear-reproduction residual above which a marker
                             falls back to exact-MLS, default 1e-4 */
   int32_t basis;         /* size m of the MLS basis p (Section 2, text after Eq. 2: Pascal's

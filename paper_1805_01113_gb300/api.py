@@ -72,7 +72,7 @@ class Transfer:
 
 
 class Context:
-    """One grid + option set (mls_create)."""
+    """One grid + option set (mls_create).  `refine` is checked (0..2) and has no effect."""
 
     def __init__(self, faces, periodic, real="f32", field=None, eps=1.0, n_sub=9, brick_log2=(3, 3, 3),
                  cond_max=1e6, refine=1, residual_max=1e-4, basis=4):
