@@ -155,7 +155,7 @@ __device__ __forceinline__ void add_runs(const Dims& D, const int o[3], int n, c
                                          int64_t M, const Scale& S, int* acc, int AX, int PS, int ACC, int AY,
                                          unsigned char* tags, unsigned char tag, FT* __restrict__ f) {
   const int c0 = threadIdx.x % 3, c1 = c0 == 2 ? 0 : c0 + 1, c2 = c0 == 0 ? 2 : c0 - 1;
-  const float s0 = S.inv[c0], s1 = S.inv[c1], s2 = S.inv[c2], limit = S.limit;
+  const float s0 = S.inv[c0], s1 = S.inv[c1], s2 = S.inv[c2];
   for (int t = threadIdx.x; t < 3 * n; t += NT) {
     const int cz = (t >= n) + (t >= 2 * n);
     const Run r(runs[t - cz * n]);
@@ -197,6 +197,7 @@ __device__ __forceinline__ void add_runs(const Dims& D, const int o[3], int n, c
     }
     // What a node with a term out of the limit added is taken back, and its terms
     // go to f.
+    const float limit = S.limit;
     if (!(most < limit)) {
       for (int k = 0; k < 9; ++k) {
         const float4 pk = phi_group<QUAD>(plane + k * cap, left);
