@@ -34,23 +34,23 @@ __device__ __forceinline__ void stage(float* dst, const __nv_bfloat16* src) {
 }
 
 // The rows with the tag, of all three components, from the field into the brick
-// (AccShape; the work is split as in flush_rows, in groups of W cells).  Cells
-// outside a walled axis, or beyond one period, belong to no support and are left
-// out.
+// (AccShape; the work is split as in flush_rows, in groups of W cells; pairs take
+// the halo cells with them).  Cells outside a walled axis, or beyond one period,
+// belong to no support and are left out.
 template <typename FT, int W, int LX, int NT>
 __device__ __forceinline__ void stage_rows(const Dims& D, const int o[3], const AccShape& A, float* brick,
                                            const unsigned char* tags, unsigned char tag, const FT* __restrict__ u) {
   constexpr int TX = 1 << LX;
-  constexpr int GROUPS = W > 1 ? TX / W : 0, CELLS = W > 1 ? 2 : TX + 2;
+  constexpr int GROUPS = W == 4 ? TX / 4 : W == 2 ? TX / 2 + 2 : 0, CELLS = W == 4 ? 2 : W == 2 ? 0 : TX + 2;
   const int rows = A.AY * A.AZ;
   const int64_t N = (int64_t)D.n[0] * D.n[1] * D.n[2];
   for (int e = threadIdx.x; e < (GROUPS + CELLS) * rows; e += NT) {
-    const bool group = W > 1 && e < GROUPS * rows;
+    const bool group = CELLS == 0 || (W > 1 && e < GROUPS * rows);
     const int s = group ? e : e - GROUPS * rows;
-    const int row = group ? s / (W > 1 ? GROUPS : 1) : s / CELLS, q = s - row * (group ? GROUPS : CELLS);
+    const int row = group ? s / (GROUPS ? GROUPS : 1) : s / (CELLS ? CELLS : 1), q = s - row * (group ? GROUPS : CELLS);
     if (tags[row] != tag) continue;
     const int ey = row % A.AY, ez = row / A.AY;
-    const int x = group ? W * q : W > 1 ? (q == 0 ? -1 : TX) : q - 1;
+    const int x = W == 2 ? 2 * q - 2 : group ? 4 * q : W == 4 ? (q == 0 ? -1 : TX) : q - 1;
     int gx = o[0] + x;
     if (gx < 0 || gx >= D.n[0]) {
       if (!D.periodic[0]) continue;
