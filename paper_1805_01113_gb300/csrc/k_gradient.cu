@@ -71,7 +71,7 @@ __device__ __forceinline__ void plain_sum(const AxisSlopes<R> f[3], const FT* __
 
 // The sums in double precision, node by node for all components at once: the
 // contraction below has a quarter more operations, and FP64 units are what this
-// form waits for (436 us on 261 120 markers in 128^3; contracted, a sixth more).
+// form waits for (433 us on 261 120 markers in 128^3; contracted, a sixth more).
 // The field is taken relative to a mean of the home cell and its six neighbours,
 // which leaves less to round than the home cell's own value where the field varies
 // from cell to cell (48^3, up to 16 waves per box: 3.4 against 4.0e-16).

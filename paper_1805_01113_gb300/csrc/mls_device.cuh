@@ -339,11 +339,11 @@ __device__ __forceinline__ void axis_slopes(const AxisNodes<R>& s, const AxisFor
     nc[a] = f.e0[a] * c[a];
     c3 += nc[a] * c[a] * c[a];
   }
-  const R bh = beta * inv_h, dg = (beta - (R(1) + beta * f.g * c3) * f.iv) * inv_h;
+  const R bh = beta * inv_h, bg = bh * f.g, dg = (beta - (R(1) + beta * f.g * c3) * f.iv) * inv_h;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     d0[a] = bh * nc[a];
-    d1[a] = -(bh * (nc[a] * c[a] - f.e0[a] * f.v) * f.g + nc[a] * dg);
+    d1[a] = -(bg * (nc[a] * c[a] - f.e0[a] * f.v) + nc[a] * dg);
   }
 }
 
