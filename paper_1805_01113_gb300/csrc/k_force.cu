@@ -1,7 +1,7 @@
 // Direct forcing (Section 2, text after Eq. 6 and Eq. 7): U_l = sum_k phi_k^l u_k,
 // F_l = (V_b,l - U_l) / dt, f_k += sum_l c_l phi_k^l F_l.  In single precision
-// one pass over the tiles; as interpolation (forming F) and spread where a tile's
-// two bricks do not fit a block, f shares memory with u, or f is bfloat16: the
+// one pass over the tiles; as interpolation (forming F) and spread where the tiles
+// are large (tiles_configure), f shares memory with u, or f is bfloat16: the
 // pass adds a tile to f every 256 markers and the spread every 512, and each
 // addition rounds to 8 bits (2.1 against 2.0e-3 of f on 2.56 M markers in 512^3).
 #include "transfer_common.cuh"

@@ -89,20 +89,21 @@ static int tile_pass_smem(int lx, int ly, int lz, bool spread) {
 // with the blocks that fit, 187 with twice, 161 with ten times as many.)
 // Bound by the shared-memory pipe (81 loads a marker and, with SPREAD, as many
 // atomics and conversions) and a tile's chain of phases.  In microseconds,
-// against the gather through L1 by runs of markers that it replaced, and against
+// against the gather through L1 by runs of markers (k_interp_runs), and against
 // that gather and the spread: 55 040 markers in 64^3 8.3 (12.3), forcing 15.1
 // (26.9); 1.04 M in 200^3 46 (49), 110 (129); 2.72 M in 256^3 97 (126), 262 (306);
 // 4 M in a 512^3 channel 161 (174), 407 (509), of which the bytes take 79 and 166;
 // 32 M in 1024^3 1 250 (1 235), 3 010 (3 390).  By runs the gathers of a warp fall
-// in few L1 sets where rows are a multiple of 128 bytes; they were faster by up to
-// 15 % on some boxes between (280 000 markers in 200^3: 17.5, now 20.2).  Runs
+// in few L1 sets where rows are a multiple of 128 bytes; they are faster by up to
+// 15 % on some boxes between (280 000 markers in 200^3: 17.5, here 20.2).  Runs
 // gathered from the staged rows took 278 in the channel: listing them costs more
 // than it saves.
-template <bool SPREAD> constexpr int kTileThreads = SPREAD ? 256 : 128;
+// Blocks have 128 threads, and 256 where they spread tiles of 2^9 cells or more,
+// which hold enough markers for that.
 constexpr int kTileWaves = 10;   // blocks per resident block
 
-template <typename FT, int W, bool SPREAD, int LX, int LY = 0, int LZ = 0>
-__global__ void __launch_bounds__(kTileThreads<SPREAD>, SPREAD ? 4 : 12) k_tile_pass(Dims D, Tiles tl, const float* __restrict__ phi,
+template <typename FT, int W, bool SPREAD, int NT, int LX, int LY = 0, int LZ = 0>
+__global__ void __launch_bounds__(NT, (SPREAD ? 1024 : 1536) / NT) k_tile_pass(Dims D, Tiles tl, const float* __restrict__ phi,
                                                               const float* __restrict__ cl,
                                                               const int32_t* __restrict__ home,
                                                               const int32_t* __restrict__ perm,
@@ -113,7 +114,6 @@ __global__ void __launch_bounds__(kTileThreads<SPREAD>, SPREAD ? 4 : 12) k_tile_
                                                               int64_t cap, int resident,
                                                               InterpOut<float, FT> io, FT* __restrict__ f) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int NT = kTileThreads<SPREAD>;
   const int ly = LY ? LY : tl.l[1], lz = LZ ? LZ : tl.l[2];
   const AccShape A(LX, ly, lz);
   float* brick = reinterpret_cast<float*>(smem_raw);
@@ -246,16 +246,26 @@ __global__ void __launch_bounds__(kTileThreads<SPREAD>, SPREAD ? 4 : 12) k_tile_
   }
 }
 
+template <typename FT, int W, bool SPREAD, int NT>
+static const void* tile_kernel_of(const int l[3]) {
+  if (l[0] == 3 && l[1] == 3 && l[2] == 3) return (const void*)k_tile_pass<FT, W, SPREAD, NT, 3, 3, 3>;
+  if (l[0] == 3 && l[1] == 3 && l[2] == 2) return (const void*)k_tile_pass<FT, W, SPREAD, NT, 3, 3, 2>;
+  switch (l[0]) {
+    case 1: return (const void*)k_tile_pass<FT, W == 4 ? 2 : W, SPREAD, NT, 1>;
+    case 2: return (const void*)k_tile_pass<FT, W, SPREAD, NT, 2>;
+    case 3: return (const void*)k_tile_pass<FT, W, SPREAD, NT, 3>;
+    case 4: return (const void*)k_tile_pass<FT, W, SPREAD, NT, 4>;
+    default: return (const void*)k_tile_pass<FT, W, SPREAD, NT, 5>;
+  }
+}
+
+static int tile_threads(const int l[3], bool spread) { return spread && l[0] + l[1] + l[2] >= 9 ? 256 : 128; }
+
 template <typename FT, int W, bool SPREAD>
 static const void* tile_kernel(const int l[3]) {
-  if (l[0] == 3 && l[1] == 3 && l[2] == 3) return (const void*)k_tile_pass<FT, W, SPREAD, 3, 3, 3>;
-  switch (l[0]) {
-    case 1: return (const void*)k_tile_pass<FT, W == 4 ? 2 : W, SPREAD, 1>;
-    case 2: return (const void*)k_tile_pass<FT, W, SPREAD, 2>;
-    case 3: return (const void*)k_tile_pass<FT, W, SPREAD, 3>;
-    case 4: return (const void*)k_tile_pass<FT, W, SPREAD, 4>;
-    default: return (const void*)k_tile_pass<FT, W, SPREAD, 5>;
-  }
+  if constexpr (SPREAD)
+    if (tile_threads(l, true) == 256) return tile_kernel_of<FT, W, true, 256>(l);
+  return tile_kernel_of<FT, W, SPREAD, 128>(l);
 }
 
 // One pass for direct forcing exists for float fields only (launch_direct_forcing).
@@ -279,17 +289,21 @@ static int copy_width(const mls_ctx* ctx, const void* u) {
   return w == 4 && ctx->tiles.l[0] < 2 ? 2 : w;
 }
 
+// Tiles of 2^8 and 2^9 cells, and for direct forcing smaller ones too.  Larger ones
+// leave few blocks per SM: 2.56 M markers in 512^3 take 125 and 128 us in tiles of
+// (3,3,3) and (3,3,2), 202 in (4,3,3), 207 in (4,4,3) and 223 in (5,3,3), by runs
+// 134 to 156 in all; direct forcing 348 and 305, 398, 490 and 510, in two kernels
+// 387 and 416, 398, 437 and 432.  In (3,2,2) 155 (150), direct forcing 369 (483).
 cudaError_t tiles_configure(mls_ctx* ctx) {
   ctx->tile_grid[0] = ctx->tile_grid[1] = 0;
-  if (ctx->opt.real == MLS_F64) return cudaSuccess;
+  const int cells = ctx->tiles.l[0] + ctx->tiles.l[1] + ctx->tiles.l[2];
+  if (ctx->opt.real == MLS_F64 || cells > 9) return cudaSuccess;
   cudaError_t e;
-  int optin = 0, sms = 0;
-  if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device)) != cudaSuccess ||
-      (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device)) != cudaSuccess)
-    return e;
-  for (int spread = 0; spread < 2; ++spread) {   // one brick fits whatever spread_tile_fits passes
+  int sms = 0;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device)) != cudaSuccess) return e;
+  for (int spread = 0; spread < 2; ++spread) {
     const int smem = tile_pass_smem(ctx->tiles.l[0], ctx->tiles.l[1], ctx->tiles.l[2], spread != 0);
-    if (smem > optin - 1024) continue;
+    if (!spread && cells < 8) continue;
     if (spread && ctx->opt.field == MLS_BF16) continue;
     int least = 64;
     for (int width = 1; width <= 4; width *= 2) {
@@ -297,7 +311,7 @@ cudaError_t tiles_configure(mls_ctx* ctx) {
       int per_sm = 0;
       if ((e = raise_smem_limit(k, smem)) != cudaSuccess ||
           (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-               &per_sm, k, spread ? kTileThreads<true> : kTileThreads<false>, smem)) != cudaSuccess)
+               &per_sm, k, tile_threads(ctx->tiles.l, spread != 0), smem)) != cudaSuccess)
         return e;
       least = std::min(least, per_sm);
     }
@@ -323,7 +337,7 @@ static cudaError_t launch_tiles_of(const mls_ctx* ctx, const mls_transfer* T, co
   const int64_t most = std::max<int64_t>(ctx->tile_grid[f ? 1 : 0], M / 1024);
   const unsigned grid = (unsigned)std::min<int64_t>(most, std::max<int64_t>(152, M / (f ? 64 : 48)));
   return cudaLaunchKernel(tile_kernel(ctx, width, f != nullptr), dim3(grid),
-                          dim3(f ? kTileThreads<true> : kTileThreads<false>), args, tile_pass_smem(tl.l[0], tl.l[1], tl.l[2], f != nullptr), s);
+                          dim3(tile_threads(tl.l, f != nullptr)), args, tile_pass_smem(tl.l[0], tl.l[1], tl.l[2], f != nullptr), s);
 }
 
 cudaError_t launch_tiles(const mls_ctx* ctx, const mls_transfer* T, const void* u, const void* Vb, double dt, void* U,

@@ -46,7 +46,7 @@ struct mls_ctx {
   // Persistent grid of the spreading kernel (blocks resident on the device).
   int spread_grid;
   int spread_threads;
-  int tile_grid[2];      // most blocks of the tile passes: gather, and gather and spread (0: its bricks do not fit)
+  int tile_grid[2];      // most blocks of the tile passes: gather, and gather and spread (0: not used)
   int collision_grid;    // persistent grid of the collision detection
   int sort_grid;         // persistent grid of the in-tile sort by home cell (0: tiles too large, no sort)
   void* refine_ws;       // refinement workspace (grown on demand)
@@ -97,6 +97,7 @@ constexpr int kBlockF64 = 64;         // the same for the double-precision build
                                       // small workloads should spread over many SMs)
 constexpr int kSpreadThreads = 128;   // threads per block of the spreading kernel
 constexpr int kTableRow = 28;         // fast-MLS table row: 27 shape-function values + 1 pad (16-byte rows)
+constexpr int kInterpThreads = 128;   // threads per block of the interpolation by runs
 constexpr int kSortThreads = 256;     // threads per block of the in-tile sort (a warp per tile)
 constexpr int kSortCellsLog2 = 12;    // tiles of up to 2^12 cells are sorted by home cell
 
@@ -186,8 +187,8 @@ cudaError_t launch_interp_gradient(const mls_ctx* ctx, const mls_transfer* T, co
 // may then be nullptr).
 cudaError_t launch_interp(const mls_ctx* ctx, const mls_transfer* T, const void* u, void* U, cudaStream_t s,
                           const void* Vb = nullptr, double dt = 0.0, void* F = nullptr);
-// The same by tiles, single precision; with f (tile_grid[1] > 0) also the
-// spreading of F in the same pass.
+// The same by tiles, single precision, where tile_grid[0] > 0; with f
+// (tile_grid[1] > 0) also the spreading of F in the same pass.
 cudaError_t launch_tiles(const mls_ctx* ctx, const mls_transfer* T, const void* u, const void* Vb, double dt, void* U,
                          void* F, void* f, cudaStream_t s);
 cudaError_t tiles_configure(mls_ctx* ctx);

@@ -2,7 +2,8 @@
 // of a home cell next to each other, and markers of one cell share their 27
 // support nodes.  A run is the markers of one home cell inside one aligned
 // group of four stored markers, so a thread that owns a run reads phi_k of its
-// group with one 16-byte load and adds a node's terms once for the whole run.
+// group with one 16-byte load and each node's field, or adds its terms, once for
+// the whole run.
 // On the workloads here a run holds 1.8 (1 280-face bodies) to 2.4 (mixed
 // bodies) markers; any order of the markers is correct, unsorted ones only
 // make shorter runs.
@@ -86,5 +87,43 @@ __device__ __forceinline__ float4 phi_group(const float* __restrict__ p, int64_t
   if constexpr (QUAD) return __ldg(reinterpret_cast<const float4*>(p));
   return make_float4(p[0], left > 1 ? p[1] : 0.f, left > 2 ? p[2] : 0.f, left > 3 ? p[3] : 0.f);
 }
+
+// U = sum_k phi_k u_k of the four markers of an aligned group whose member(s)
+// of home cell i form a run (the other components of the result are not
+// theirs): each node's velocity is read once for the whole run.
+template <typename FT, bool QUAD>
+__device__ __forceinline__ void gather_run(const Dims& D, const int i[3], const FT* __restrict__ u,
+                                           const float* __restrict__ plane, int64_t cap, int64_t left, float4 U[3]) {
+  const int64_t N = (int64_t)D.n[0] * D.n[1] * D.n[2];
+  int xs[3], ys[3], zs[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    xs[a] = wrap(i[0] + a - 1, D.n[0], D.periodic[0]);
+    ys[a] = wrap(i[1] + a - 1, D.n[1], D.periodic[1]);
+    zs[a] = wrap(i[2] + a - 1, D.n[2], D.periodic[2]);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) U[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int cz = 0; cz < 3; ++cz)
+#pragma unroll
+    for (int cy = 0; cy < 3; ++cy) {
+      const FT* ur = u + (int64_t)((zs[cz] * D.n[1] + ys[cy]) * D.n[0]);   // below n_x n_y n_z < 2^31
+#pragma unroll
+      for (int cx = 0; cx < 3; ++cx) {
+        const float4 p = phi_group<QUAD>(plane + (9 * cz + 3 * cy + cx) * cap, left);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const float v = load_field<float, FT>(ur + q * N + xs[cx]);
+          U[q].x += p.x * v;
+          U[q].y += p.y * v;
+          U[q].z += p.z * v;
+          U[q].w += p.w * v;
+        }
+      }
+    }
+}
+
+__device__ __forceinline__ float at(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
 
 }  // namespace mls
