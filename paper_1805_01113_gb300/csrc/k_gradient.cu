@@ -63,7 +63,7 @@ __device__ __forceinline__ void plain_sum(const AxisSlopes<R> f[3], const FT* __
 #pragma unroll
     for (int q = 0; q < 9; ++q)
       if (q == k / 3) o += rows[q / 3][q % 3];
-    const R v = field_value<R, FT>(u + o);
+    const R v = load_field<R, FT>(u + o);
 #pragma unroll
     for (int d = 0; d < 3; ++d) out[d] += w[d] * v;
   }
@@ -81,7 +81,7 @@ __device__ __forceinline__ void node_sum(const AxisSlopes<double> f[3], const FT
   double mid[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    auto at = [&](int x, int y, int z) { return field_value<double, FT>(u + c * N + rows[z][y] + xs[x]); };
+    auto at = [&](int x, int y, int z) { return load_field<double, FT>(u + c * N + rows[z][y] + xs[x]); };
     const double own = at(1, 1, 1);
     mid[c] = 0.125 * (((at(0, 1, 1) + at(2, 1, 1)) + (at(1, 0, 1) + at(1, 2, 1))) +
                       ((at(1, 1, 0) + at(1, 1, 2)) + (own + own)));
@@ -103,7 +103,7 @@ __device__ __forceinline__ void node_sum(const AxisSlopes<double> f[3], const FT
         const double w[3] = {f[0].d0[cx] * k1 + f[0].d1[cx] * k0, e0 * ky1 + e1 * ky0, e0 * kz1 + e1 * kz0};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const double v = field_value<double, FT>(u + c * N + rows[cz][cy] + xs[cx]) - mid[c];
+          const double v = load_field<double, FT>(u + c * N + rows[cz][cy] + xs[cx]) - mid[c];
 #pragma unroll
           for (int d = 0; d < 3; ++d) out[c][d] += w[d] * v;
         }
@@ -182,8 +182,8 @@ __global__ void __launch_bounds__(kGradThreads<R>, sizeof(R) == 4 ? 4 : 1)
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
         const FT* ur = uc + rows[cz][b];
-        v[b] = field_value<R, FT>(ur + xs[1]);
-        const R lo = field_value<R, FT>(ur + xs[0]) - v[b], hi = field_value<R, FT>(ur + xs[2]) - v[b];
+        v[b] = load_field<R, FT>(ur + xs[1]);
+        const R lo = load_field<R, FT>(ur + xs[0]) - v[b], hi = load_field<R, FT>(ur + xs[2]) - v[b];
         e0[b] = ends(f[0].e0, lo, hi);
         e1[b] = ends(f[0].e1, lo, hi);
         d0[b] = ends(f[0].d0, lo, hi);

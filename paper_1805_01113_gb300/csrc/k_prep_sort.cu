@@ -52,7 +52,7 @@ cudaError_t launch_prep(int real, const void* V, int64_t nv, const int32_t* tri,
 // fill the GPU several times over (their loads then overlap), 1 on small ones
 // (which need every block they can get).
 constexpr int kLocatePer = 4;
-inline int locate_per(int64_t M) { return M >= (int64_t)kLocatePer * 152 * 2048 ? kLocatePer : 1; }
+inline int locate_per(int64_t M) { return M >= (int64_t)kLocatePer * kSMs * 2048 ? kLocatePer : 1; }
 
 // Triangles whose markers the locate kernel forms itself (the preparation
 // fused into it): vertices, their count, the triangles, and where the

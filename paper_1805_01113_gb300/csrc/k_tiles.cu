@@ -35,8 +35,9 @@ __device__ __forceinline__ void stage(float* dst, const __nv_bfloat16* src) {
 
 // The rows with the tag, of all three components, from the field into the brick
 // (AccShape; the work is split as in flush_rows, in groups of W cells; pairs take
-// the halo cells with them).  Cells outside a walled axis, or beyond one period,
-// belong to no support and are left out.
+// the halo cells with them).  Cells and rows outside a walled axis, or beyond one
+// period, belong to no support and are left out: a row can carry an equal tag of
+// 255 tiles ago.
 template <typename FT, int W, int LX, int NT>
 __device__ __forceinline__ void stage_rows(const Dims& D, const int o[3], const AccShape& A, float* brick,
                                            const unsigned char* tags, unsigned char tag, const FT* __restrict__ u) {
@@ -57,9 +58,10 @@ __device__ __forceinline__ void stage_rows(const Dims& D, const int o[3], const 
       gx = gx < 0 ? gx + D.n[0] : gx - D.n[0];
       if (gx < 0 || gx >= D.n[0]) continue;
     }
+    const int gy = wrap(o[1] - 1 + ey, D.n[1], D.periodic[1]), gz = wrap(o[2] - 1 + ez, D.n[2], D.periodic[2]);
+    if (gy >= D.n[1] || gz >= D.n[2]) continue;
     float* a = brick + AccShape::kFront + ez * A.PS + ey * A.AX + x;
-    const FT* ur = u + (int64_t)((wrap(o[2] - 1 + ez, D.n[2], D.periodic[2]) * D.n[1] +
-                                  wrap(o[1] - 1 + ey, D.n[1], D.periodic[1])) * D.n[0] + gx);
+    const FT* ur = u + (int64_t)((gz * D.n[1] + gy) * D.n[0] + gx);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       if (group)
@@ -335,7 +337,7 @@ static cudaError_t launch_tiles_of(const mls_ctx* ctx, const mls_transfer* T, co
                   (void*)&T->n_items, (void*)&T->offsets, (void*)&T->counts, &M, &cap, &resident, &io, &f};
   const int wu = copy_width(ctx, u), width = f && wu == 4 && !spread_vec_aligned(ctx, f) ? 2 : wu;
   const int64_t most = std::max<int64_t>(ctx->tile_grid[f ? 1 : 0], M / 1024);
-  const unsigned grid = (unsigned)std::min<int64_t>(most, std::max<int64_t>(152, M / (f ? 64 : 48)));
+  const unsigned grid = (unsigned)std::min<int64_t>(most, std::max<int64_t>(kSMs, M / (f ? 64 : 48)));
   return cudaLaunchKernel(tile_kernel(ctx, width, f != nullptr), dim3(grid),
                           dim3(tile_threads(tl.l, f != nullptr)), args, tile_pass_smem(tl.l[0], tl.l[1], tl.l[2], f != nullptr), s);
 }

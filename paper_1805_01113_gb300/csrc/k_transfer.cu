@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kInterpThreads, 8) k_interp_runs(Dims D, const
 // 0.70 ms and 87 us for the bytes: issue (39 % active), the shared-memory pipe
 // and the waits between a tile's phases share the rest, at 28 warps per SM.  A
 // thread per marker issuing its own 81 atomics, chunks of 128 markers, took
-// 2.06 ms and 318 us, with three times the error against double precision.
+// 2.06 ms and 318 us.
 template <typename FT, bool VEC, int LX, int LY = 0, int LZ = 0>
 __global__ void __launch_bounds__(kSpreadThreads, 8) k_spread(Dims D, Tiles tl, const float* __restrict__ phi,
                                                            const float* __restrict__ cl,

@@ -92,6 +92,7 @@ namespace mls {
 
 constexpr int kScanTile = 4096;       // bins per scan tile
 constexpr int kScanMaxTiles = 8192;   // bins <= 32 Mi
+constexpr int kSMs = 152;             // multiprocessors of a GB300, where a rule needs them without a device query
 constexpr int kBlock = 256;           // threads per block of the per-marker kernels
 constexpr int kBlockF64 = 64;         // the same for the double-precision builds and gradient (FP64-bound:
                                       // small workloads should spread over many SMs)
@@ -107,7 +108,7 @@ constexpr int kSortCellsLog2 = 12;    // tiles of up to 2^12 cells are sorted by
 // One sphere of 5 120 markers, double precision, a whole step: 84 -> 76 us.
 inline unsigned block_threads(int64_t n, int most) {
   int t = most;
-  while (t > 32 && (n + t - 1) / t < 2 * 152) t /= 2;
+  while (t > 32 && (n + t - 1) / t < 2 * kSMs) t /= 2;
   return (unsigned)t;
 }
 inline unsigned blocks_for(int64_t n, unsigned threads) { return (unsigned)((n + threads - 1) / threads); }
